@@ -38,16 +38,69 @@ __device__ __forceinline__ double rdotv(int q, const double u[3]) {
 __device__ __forceinline__ double rdot3(const double a[3], const double b[3]) {
   return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
+// u.u of a vector of D components: the squares of the absent ones, +0, change
+// no sum of squares
+template <int D>
+__device__ __forceinline__ double rsq(const double u[3]) {
+  double s = u[0] * u[0];
+#pragma unroll
+  for (int d = 1; d < D; d++) s = s + u[d] * u[d];
+  return s;
+}
 
 template <class L>
 __device__ __forceinline__ double reta(int q, double phi, double k0) {
   return q == 0 ? 1.0 + k0 * (1.0 - phi) : phi;
 }
 
+// Division by the two lattice constants.  cs2 = RN(1/3) = (1 - 2^-54)/3 and
+// two_cs4 = RN(2 cs2 cs2) = (2/9)(1 - 2^-54), so x / cs2 = 3 x (1 + 2^-54 +
+// ...) and x / two_cs4 = 4.5 x (1 + 2^-54 + ...): one fused multiply-add with
+// the correction x c 2^-54 (c = 3, 4.5; c x 2^-54 is rounded once) rounds
+// to the same double as the division.  (Division by a constant known in
+// advance, after Brisebarre, Muller and Raina, "Accelerating correctly
+// rounded floating-point division when the divisor is known in advance",
+// IEEE Trans. Comput. 53, 2004.  c x has at most 2 (4) bits below the
+// result's last place, so its fraction of that place is a multiple of 1/4
+// (1/16); the correction lies in [1/4, 1/2) of it, and the sums that come
+// within a last place of a tie need c x = (2^52 + 1/4) u, (3 2^51 + 1/8) u
+// or (2^52 + 1/4) u with u four, four or eight places of x, none of which is
+// c times an integer.)  It holds while the correction is not rounded at
+// the underflow threshold, |x| >= 2^-963, and for x = 0; ref_plain_div
+// decides that per node.  FP64 is the step's bound: a division costs two
+// operations instead of the nine or more of the IEEE sequence, and 44 of
+// a D2Q9 node's divisions are by these constants.
+static_assert(CS2 == 0x1.5555555555555p-2 && 2.0 * CS2 * CS2 == 0x1.c71c71c71c71cp-3,
+              "the multipliers below are those of RN(1/3) and RN(2/9 (1 - 2^-54))");
 struct RefConst {
   double cs2, two_cs4, k0;
 };
+template <bool FAST>
+__device__ __forceinline__ double div_cs2(double x, const RefConst &k) {
+  return FAST ? __fma_rn(x, 3.0, __dmul_rn(x, 3.0 * 0x1p-54)) : x / k.cs2;
+}
+template <bool FAST>
+__device__ __forceinline__ double div_two_cs4(double x, const RefConst &k) {
+  return FAST ? __fma_rn(x, 4.5, __dmul_rn(x, 4.5 * 0x1p-54)) : x / k.two_cs4;
+}
+// May a component be neither zero nor at least 2^-300 in magnitude?  When
+// no component of a vector is, every v.u and (v.u)^2 - cs2 u.u of it is zero
+// or at least 2^-757, in range of the two forms above.  (Magnitudes whose
+// high word is zero pass: below 2^-1042 the product 3 x is exact, a tie-free
+// subnormal, and the squares vanish.)
+__device__ __forceinline__ bool ref_small(double x) {
+  const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  return h - 1u < ((1023u - 300u) << 20) - 1u;
+}
+template <int D>
+__device__ __forceinline__ bool ref_plain_div(const double u[3]) {
+  bool s = false;
+#pragma unroll
+  for (int d = 0; d < D; d++) s = s || ref_small(u[d]);
+  return s;
+}
 
+// The literal forms (initial state, face rules)
 template <class L>
 __device__ __forceinline__ double rfeqI(int q, const RefConst &k, double phi, double eps, const double u[3]) {
   const double vu = rdotv<L>(q, u), uu = rdot3(u, u);
@@ -58,12 +111,18 @@ __device__ __forceinline__ double rfeqS(int q, const RefConst &k, double alpha, 
   const double vu = rdotv<L>(q, u), uu = rdot3(u, u);
   return L::w(q) * alpha * (1.0 + vu / k.cs2 + (vu * vu - k.cs2 * uu) / k.two_cs4);
 }
-template <class L>
-__device__ __forceinline__ double rfeqL(int q, const RefConst &k, double psi, double S, const double G[3]) {
-  return L::w(q) * (S * reta<L>(q, psi, k.k0) + rdotv<L>(q, G) / k.cs2);
-}
 
-__device__ __forceinline__ double spalB(double x) { return x <= 0.0 ? 0.0 : (x >= 1.0 ? 1.0 : x); }
+// Comparisons on the bits (a comparison in double takes the FP64 pipe): x > y
+// for y >= 0, false for NaN; the clamp to [0, 1], NaN kept.
+__device__ __forceinline__ bool ref_above(double x, double y) {
+  const long long b = __double_as_longlong(x);
+  return b > __double_as_longlong(y) && b <= 0x7ff0000000000000LL;
+}
+__device__ __forceinline__ double spalB(double x) {
+  const long long b = __double_as_longlong(x);
+  if ((b & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL) return x;
+  return b <= 0 ? 0.0 : (b >= 0x3ff0000000000000LL ? 1.0 : x);
+}
 
 // Per-node macroscopic state of the reference path.
 struct RefMom {
@@ -76,37 +135,44 @@ struct RefMom {
 template <class L>
 __device__ __forceinline__ void ref_moments(const StepArgs &a, const double f[6][L::Q], RefMom &m) {
   constexpr int D = L::D;
-  m.eps_g = m.eps_l = m.a_g = m.a_l = m.b_g = m.b_l = 0.0;
+  // sums in lexicographic order, each from its first term (0 + x is x)
+  double *const z[6] = {&m.eps_g, &m.eps_l, &m.a_g, &m.a_l, &m.b_g, &m.b_l};
+#pragma unroll
+  for (int s = 0; s < 6; s++) {
+    *z[s] = f[s][0];
+#pragma unroll
+    for (int q = 1; q < L::Q; q++) *z[s] += f[s][q];
+  }
+  auto signed_sum = [&](const double *fs, auto coef) {
+    double r = 0.0;
+    bool first = true;
+#pragma unroll
+    for (int q = 1; q < L::Q; q++) {
+      const int c = coef(q);
+      if (c != 0) {
+        const double t = c > 0 ? fs[q] : -fs[q];
+        r = first ? t : r + t;
+        first = false;
+      }
+    }
+    return r;
+  };
 #pragma unroll
   for (int d = 0; d < 3; d++) {
-    m.u_g[d] = m.u_l[d] = m.J_g[d] = m.J_l[d] = 0.0;
+    auto v = [d](int q) { return L::v(q, d); };
+    m.u_g[d] = d < D ? signed_sum(f[0], v) : 0.0;
+    m.u_l[d] = d < D ? signed_sum(f[1], v) : 0.0;
+    m.J_g[d] = d < D ? signed_sum(f[2], v) : 0.0;
+    m.J_l[d] = d < D ? signed_sum(f[3], v) : 0.0;
 #pragma unroll
-    for (int e = 0; e < 3; e++) m.Pi_g[d][e] = m.Pi_l[d][e] = 0.0;
-  }
-#pragma unroll
-  for (int q = 0; q < L::Q; q++) {
-    m.eps_g += f[0][q];
-    m.eps_l += f[1][q];
-    m.a_g += f[2][q];
-    m.a_l += f[3][q];
-    m.b_g += f[4][q];
-    m.b_l += f[5][q];
-#pragma unroll
-    for (int d = 0; d < D; d++) {
-      const int vd = L::v(q, d);
-      if (vd != 0) {
-        m.u_g[d] += vd > 0 ? f[0][q] : -f[0][q];
-        m.u_l[d] += vd > 0 ? f[1][q] : -f[1][q];
-        m.J_g[d] += vd > 0 ? f[2][q] : -f[2][q];
-        m.J_l[d] += vd > 0 ? f[3][q] : -f[3][q];
-      }
-#pragma unroll
-      for (int e = 0; e < D; e++) {
-        const int ve = L::v(q, d) * L::v(q, e);
-        if (ve != 0) {
-          m.Pi_g[d][e] += ve > 0 ? f[0][q] : -f[0][q];
-          m.Pi_l[d][e] += ve > 0 ? f[1][q] : -f[1][q];
-        }
+    for (int e = 0; e < 3; e++) {
+      auto vv = [d, e](int q) { return L::v(q, d) * L::v(q, e); };
+      if (e < d) {
+        m.Pi_g[d][e] = m.Pi_g[e][d];
+        m.Pi_l[d][e] = m.Pi_l[e][d];
+      } else {
+        m.Pi_g[d][e] = e < D ? signed_sum(f[0], vv) : 0.0;
+        m.Pi_l[d][e] = e < D ? signed_sum(f[1], vv) : 0.0;
       }
     }
   }
@@ -116,7 +182,7 @@ __device__ __forceinline__ void ref_moments(const StepArgs &a, const double f[6]
     m.al_l = m.a_l;
   } else {
     const double Bg = spalB(m.a_g), Bl = spalB(m.a_l);
-    m.al_g = (Bg + Bl > 0.0) ? Bg / (Bg + Bl) : 0.5;
+    m.al_g = ref_above(Bg + Bl, 0.0) ? Bg / (Bg + Bl) : 0.5;
     m.al_l = 1.0 - m.al_g;
   }
 }
@@ -155,7 +221,7 @@ __global__ void __launch_bounds__(256) k_step_ref(const StepArgs a) {
     load_node<L, double, double>(a, g, a.parity, P);
     ref_moments<L>(a, f, m);
 #pragma unroll
-    for (int d = 0; d < 3; d++) {
+    for (int d = 0; d < D; d++) {
       c_g[d] = m.al_l * (m.u_g[d] - m.u_l[d]);  // Eq. (velocitybeta), beta = 1
       c_l[d] = m.al_g * (m.u_l[d] - m.u_g[d]);
     }
@@ -186,8 +252,8 @@ __global__ void __launch_bounds__(256) k_step_ref(const StepArgs a) {
   double *held = (double *)a.held;
   double Spp_g, Spp_l, Lam;
   if (a.latch) {
-    Spp_g = S_g - a.gamma * rdot3(m.u_g, m.u_g) * (m.eps_g - 1.0);
-    Spp_l = S_l - a.gamma * rdot3(m.u_l, m.u_l) * (phi * m.eps_l - 1.0);
+    Spp_g = S_g - a.gamma * rsq<D>(m.u_g) * (m.eps_g - 1.0);
+    Spp_l = S_l - a.gamma * rsq<D>(m.u_l) * (phi * m.eps_l - 1.0);
     Lam = m.al_g * m.al_l * (m.al_g + m.al_l * a.R);  // Eq. (Lambda)
     held[g.node] = Spp_g;
     held[a.plane + g.node] = Spp_l;
@@ -224,8 +290,9 @@ __global__ void __launch_bounds__(256) k_step_ref(const StepArgs a) {
         sg_ = a.nuef_g * (a.omega_g * (Peq_g - m.Pi_g[d][e]) + a.psi_g * K.cs2 * Spp_g);
         sl_ = a.nuef_l * (a.omega_l * (Peq_l - m.Pi_l[d][e]) + a.psi_l * K.cs2 * Spp_l);
       } else {
-        sg_ = (1.0 - 0.5 * a.omega_g) * (Peq_g - m.Pi_g[d][e]) - (d == e ? 0.5 * K.cs2 * a.psi_g * Spp_g : 0.0);
-        sl_ = (1.0 - 0.5 * a.omega_l) * (Peq_l - m.Pi_l[d][e]) - (d == e ? 0.5 * K.cs2 * a.psi_l * Spp_l : 0.0);
+        // A = 1 - omega/2 and B = -(cs2 psi/2), formed once on the host
+        sg_ = a.A_g * (Peq_g - m.Pi_g[d][e]) - (d == e ? -a.B_g * Spp_g : 0.0);
+        sl_ = a.A_l * (Peq_l - m.Pi_l[d][e]) - (d == e ? -a.B_l * Spp_l : 0.0);
       }
       sgg += sg_ * gG_g[e];
       slg += sl_ * gG_l[e];
@@ -237,35 +304,32 @@ __global__ void __launch_bounds__(256) k_step_ref(const StepArgs a) {
   // drag (Eqs. (interphasemomentum), (CliftGraceWeber)), wall friction
   // (Eq. (wallmomentum1D)), forces (Eqs. (Gg), (Gl), (Gg1D))
   const double KI = a.cgw ? a.kappa_I * Lam : a.kappa_I;
-  const double KW = a.cgw ? a.kappa_W * Lam : a.kappa_W;
   double du[3];
 #pragma unroll
   for (int d = 0; d < 3; d++) du[d] = m.u_l[d] - m.u_g[d];
-  const double ag_d = m.al_g > a.afloor ? m.al_g : a.afloor;
-  const double al_d = m.al_l > a.afloor ? m.al_l : a.afloor;
-  const double ndu = sqrt(rdot3(du, du)), nul = sqrt(rdot3(m.u_l, m.u_l));
+  const double ag_d = ref_above(m.al_g, a.afloor) ? m.al_g : a.afloor;
+  const double al_d = ref_above(m.al_l, a.afloor) ? m.al_l : a.afloor;
+  const double ndu = sqrt(rsq<D>(du));
   double G_g[3] = {0.0, 0.0, 0.0}, G_l[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int d = 0; d < D; d++) {
     double gg = Spp_g * m.u_g[d] + sgG[d] / ag_d;
     if (d == gax) gg = gg + a.buoy;
     G_g[d] = gg + KI * ndu * du[d] / ag_d;
-    G_l[d] = Spp_l * m.u_l[d] + slG[d] / al_d - KI * ndu * du[d] / (a.R * al_d) - KW * nul * m.u_l[d] / (a.R * al_d);
+    G_l[d] = Spp_l * m.u_l[d] + slG[d] / al_d - KI * ndu * du[d] / (a.R * al_d);
+  }
+  if (a.kappa_W != 0.0) {  // without wall friction the term is an exact zero
+    const double KW = a.cgw ? a.kappa_W * Lam : a.kappa_W;
+    const double nul = sqrt(rsq<D>(m.u_l));
+#pragma unroll
+    for (int d = 0; d < D; d++) G_l[d] = G_l[d] - KW * nul * m.u_l[d] / (a.R * al_d);
   }
 
   const double aeq_g = a.spalding == 2 ? m.al_g : m.a_g;
   const double aeq_l = a.spalding == 2 ? m.al_l : m.a_l;
   double *base = (double *)a.pop;
-#pragma unroll
-  for (int q = 0; q < Q; q++) {
-    double out[6];
-    out[0] = f[0][q] + a.omega_g * (rfeqI<L>(q, K, 1.0, m.eps_g, m.u_g) - f[0][q]) + rfeqL<L>(q, K, a.psi_g, Spp_g, G_g);
-    out[1] = f[1][q] + a.omega_l * (rfeqI<L>(q, K, phi, m.eps_l, m.u_l) - f[1][q]) + rfeqL<L>(q, K, a.psi_l, Spp_l, G_l);
-    out[2] = f[2][q] + a.omega_a * (rfeqS<L>(q, K, aeq_g, m.u_g) - f[2][q]);
-    out[3] = f[3][q] + a.omega_a * (rfeqS<L>(q, K, aeq_l, m.u_l) - f[3][q]);
-    out[4] = rfeqS<L>(q, K, 1.0, c_g);
-    out[5] = rfeqS<L>(q, K, 1.0, c_l);
-
+  // face rules of direction q and its store
+  auto finish = [&](const int q, double out[6]) {
     const bool cross = crosses<L>(g, q, +1);
     if (cross) {
       const int rule = face_rule<L>(a, g, q);
@@ -328,7 +392,69 @@ __global__ void __launch_bounds__(256) k_step_ref(const StepArgs a) {
     const long long idx = write_slot<L>(a, g, q, cross, a.parity, pq);
 #pragma unroll
     for (int s = 0; s < 6; s++) base[(long long)(s * Q + pq) * a.plane + idx] = out[s];
-  }
+  };
+
+  // Collisions, the moving directions in pairs (q, opp q): v.u of the two is
+  // equal and opposite, exactly, and so are v.u / cs2 and v.G / cs2, while
+  // ((v.u)^2 - cs2 u.u)/(2 cs2 cs2) is the same number; each is formed once,
+  // and the literal expressions around them are evaluated for either sign in
+  // their own order.  With the two-operation divisions and without the
+  // operations on exact zeros and uniform constants: 500 x 1030 nodes of D2Q9
+  // 1.43 -> 0.90 ms a step (360 -> 573 MLUPS), the FP64 pipe the bound before
+  // and after.
+  auto collide = [&](auto FASTc) {
+    constexpr bool FAST = decltype(FASTc)::value;
+    const double cug = K.cs2 * rsq<D>(m.u_g), cul = K.cs2 * rsq<D>(m.u_l);
+    const double ccg = K.cs2 * rsq<D>(c_g), ccl = K.cs2 * rsq<D>(c_l);
+    // quadratic term of a direction, and f^eq of unit alpha: (1 + a) + b
+    auto quad = [&](double vu, double cuu) { return div_two_cs4<FAST>(vu * vu - cuu, K); };
+    {
+      double out[6];
+      const double bg = quad(0.0, cug), bl = quad(0.0, cul);
+      const double wq = L::w(0);
+      out[0] = f[0][0] + a.omega_g * (wq * (m.eps_g + bg) - f[0][0]) + wq * (Spp_g * a.eta0_g);
+      out[1] = f[1][0] + a.omega_l * (wq * (m.eps_l * reta<L>(0, phi, K.k0) + bl) - f[1][0]) +
+               wq * (Spp_l * a.eta0_l);
+      out[2] = f[2][0] + a.omega_a * (wq * aeq_g * (1.0 + bg) - f[2][0]);
+      out[3] = f[3][0] + a.omega_a * (wq * aeq_l * (1.0 + bl) - f[3][0]);
+      out[4] = wq * (1.0 + quad(0.0, ccg));
+      out[5] = wq * (1.0 + quad(0.0, ccl));
+      finish(0, out);
+    }
+    const double eg = m.eps_g, el = m.eps_l * reta<L>(1, phi, K.k0);
+    const double sg = Spp_g * reta<L>(1, a.psi_g, K.k0), sl = Spp_l * reta<L>(1, a.psi_l, K.k0);
+#pragma unroll
+    for (int q = 1; q < Q; q++) {
+      const int qo = L::opp(q);
+      if (q < qo) {
+        const double wq = L::w(q), wag = wq * aeq_g, wal = wq * aeq_l;
+        const double vug = rdotv<L>(q, m.u_g), vul = rdotv<L>(q, m.u_l), vcg = rdotv<L>(q, c_g), vcl = rdotv<L>(q, c_l);
+        const double ag = div_cs2<FAST>(vug, K), al = div_cs2<FAST>(vul, K);
+        const double gg = div_cs2<FAST>(rdotv<L>(q, G_g), K), gl = div_cs2<FAST>(rdotv<L>(q, G_l), K);
+        const double cg = div_cs2<FAST>(vcg, K), cl = div_cs2<FAST>(vcl, K);
+        const double bg = quad(vug, cug), bl = quad(vul, cul), dg = quad(vcg, ccg), dl = quad(vcl, ccl);
+        double oa[6], ob[6];
+        oa[0] = f[0][q] + a.omega_g * (wq * (eg + ag + bg) - f[0][q]) + wq * (sg + gg);
+        ob[0] = f[0][qo] + a.omega_g * (wq * (eg - ag + bg) - f[0][qo]) + wq * (sg - gg);
+        oa[1] = f[1][q] + a.omega_l * (wq * (el + al + bl) - f[1][q]) + wq * (sl + gl);
+        ob[1] = f[1][qo] + a.omega_l * (wq * (el - al + bl) - f[1][qo]) + wq * (sl - gl);
+        oa[2] = f[2][q] + a.omega_a * (wag * (1.0 + ag + bg) - f[2][q]);
+        ob[2] = f[2][qo] + a.omega_a * (wag * (1.0 - ag + bg) - f[2][qo]);
+        oa[3] = f[3][q] + a.omega_a * (wal * (1.0 + al + bl) - f[3][q]);
+        ob[3] = f[3][qo] + a.omega_a * (wal * (1.0 - al + bl) - f[3][qo]);
+        oa[4] = wq * (1.0 + cg + dg);
+        ob[4] = wq * (1.0 - cg + dg);
+        oa[5] = wq * (1.0 + cl + dl);
+        ob[5] = wq * (1.0 - cl + dl);
+        finish(q, oa);
+        finish(qo, ob);
+      }
+    }
+  };
+  const bool plain_div = ref_plain_div<D>(m.u_g) || ref_plain_div<D>(m.u_l) || ref_plain_div<D>(c_g) ||
+                         ref_plain_div<D>(c_l) || ref_plain_div<D>(G_g) || ref_plain_div<D>(G_l);
+  if (plain_div) collide(std::false_type{});
+  else collide(std::true_type{});
 }
 
 // Initial equilibria (full values), Sec. 2 initial state: eps_g = p_k/cs2,

@@ -155,6 +155,24 @@ def test_fp64_reference_is_bitwise(name):
         assert np.array_equal(s.populations(sch), o.pops(sch)), (name, sch)
 
 
+@pytest.mark.parametrize("lat, dims", [("D1Q3", (40,)), ("D2Q9", (20, 13)), ("D3Q19", (9, 8, 7))])
+@pytest.mark.parametrize("scale", [0.0, 1e-88, 1e-95, 1e-300])
+def test_fp64_reference_tiny_velocities_bitwise(lat, dims, scale):
+    """Velocity components about 2^-300 and below, where a node takes the
+    literal divisions by cs2 and 2 cs2^2 (lbm_ref.cuh), beside nodes that take
+    the two-operation form, in the same warp."""
+    D = lbm.LATTICE[lat]
+    f = lbm_inputs.fields_random(D, dims, seed=3, alpha=(0.2, 0.6), u_amp=1.0, pk_amp=0.0)
+    for k in ("u_g", "u_l"):
+        f[k] = f[k] * scale
+        f[k][:, ::5] *= 1e-3 / max(scale, 1e-3)
+    p = dict(R=50.0, omega_g=0.6, omega_l=1.2, omega_alpha=1.5, g_axis=0, bc_lo=(WALL, 0, 0), bc_hi=(WALL, 0, 0))
+    for steps in (1, 6):
+        got, ref, s, o = run_pair(lat, dims, p, f, steps, "fp64")
+        for k in ("alpha_g", "u_g", "u_l", "p_k", "S_g", "S_l"):
+            assert np.array_equal(got[k], ref[k]), (k, steps)
+
+
 @pytest.mark.parametrize("name", sorted(CASES))
 def test_parity_fp64dev(name):
     """The fast kernels' deviation arithmetic, in double.  Bar 1e-9: the
