@@ -9,6 +9,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <utility>
 #include <vector>
 
 #include "../../include/lbm.h"
@@ -49,6 +50,7 @@ cudaError_t launch_ref_init_2(const MomArgs &, const double *, const double *, c
                               unsigned, cudaStream_t);
 cudaError_t launch_ref_init_3(const MomArgs &, const double *, const double *, const double *, const double *,
                               unsigned, cudaStream_t);
+cudaError_t launch_ref_steps_1d(const Ref1DArgs &, cudaStream_t);
 
 __global__ void k_diag_final(const double *partials, int nblocks, double *out) {
   // One warp per diagnostic, each lane sums a fixed strided subset, then a
@@ -144,6 +146,13 @@ static double ramp(const double mm[2], long long t, int nt) {
   return (mm[1] - mm[0]) * tanh((double)t / (double)nt) + mm[0];
 }
 
+// Inlet values at step t, Eq. (transient)
+static void inlet_at(const lbm_params &p, long long t, double &aIN, double &ugIN, double &ulIN) {
+  aIN = ramp(p.in_alpha, t, p.ramp_nt);
+  ugIN = ramp(p.in_ug, t, p.ramp_nt);
+  ulIN = p.inlet_ul_mode == 1 ? -aIN * ugIN / (1.0 - aIN) : ramp(p.in_ul, t, p.ramp_nt);
+}
+
 // Per-step arguments: everything constant plus parity, latch and inlet values.
 static StepArgs make_args(const lbm_ctx *c, long long t) {
   const lbm_params &p = c->p;
@@ -205,9 +214,7 @@ static StepArgs make_args(const lbm_ctx *c, long long t) {
   a.spalding = p.spalding_mode;
   a.r_ag = c->r_ag;
   a.r_al = c->r_al;
-  a.aIN = ramp(p.in_alpha, t, p.ramp_nt);
-  a.ugIN = ramp(p.in_ug, t, p.ramp_nt);
-  a.ulIN = p.inlet_ul_mode == 1 ? -a.aIN * a.ugIN / (1.0 - a.aIN) : ramp(p.in_ul, t, p.ramp_nt);
+  inlet_at(p, t, a.aIN, a.ugIN, a.ulIN);
   a.plain = c->prec == LBM_FP64;
   a.cfield = c->cfield;
   a.beta_own = c->cfield && c->first_step;
@@ -336,6 +343,20 @@ static int choose_tiles(lbm_ctx *c) {
   return LBM_OK;
 }
 
+// Steps per launch of a short FP64 1D lattice (lbm_ref_1d.cuh); 0: one step
+// per launch of k_step_ref.  The most steps whose blocks (smaller cores, more
+// blocks) still leave one block per SM, else two per SM: a step takes 5.3
+// and 8.8 us, a launch 5 us more (2,048 nodes: 2 steps and one block per SM
+// 8.2 us a step, 4 and two 9.7).  With more blocks k_step_ref's 12.7 us a
+// step, flat up to 8,192 nodes, is less (8,192: 20.5 with 2 steps per launch).
+static int several_steps_1d(const lbm_ctx *c) {
+  if (c->D != 1 || c->prec != LBM_FP64) return 0;
+  for (int per_sm = 1; per_sm <= 2; per_sm++)
+    for (int n = R1_MAX_STEPS; n >= per_sm; n--)
+      if ((c->N + r1_core(n) - 1) / r1_core(n) <= (long long)per_sm * c->sms) return n;
+  return 0;
+}
+
 namespace lbm {
 StepArgs ctx_step_args(const lbm_ctx *c, long long t) { return make_args(c, t); }
 cudaError_t launch_batch_step(int lattice, int prec, const StepArgs *args, const WorkItem *work, unsigned nwork,
@@ -453,6 +474,11 @@ int lbm_create(int dim, int lattice, int nx, int ny, int nz, const lbm_params *p
   c->plane = (c->N + 63) / 64 * 64;  // 256-byte aligned planes for every store type
   c->p = q;
   c->nblk_flat = (unsigned)((c->N + 255) / 256);
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || c->sms < 1)
+    c->sms = 1;  // no device: the allocations below fail
+  c->steps_1d = several_steps_1d(c);
   default_tile(c);
   int rc = choose_tiles(c);
   if (rc) { int e = rc; delete c; return e; }
@@ -460,7 +486,8 @@ int lbm_create(int dim, int lattice, int nx, int ny, int nz, const lbm_params *p
   size_t pop_bytes = store_bytes_per_dir(c->prec, nsch) * c->Q * c->plane;
   size_t held_bytes = (size_t)3 * c->plane * held_size(c->prec);
   size_t c_bytes = (size_t)4 * dim * c->plane * held_size(c->prec);
-  if (cudaMalloc(&c->pop, pop_bytes) != cudaSuccess || cudaMalloc(&c->held, held_bytes) != cudaSuccess ||
+  const size_t copies = c->steps_1d ? 2 : 1;
+  if (cudaMalloc(&c->pop, copies * pop_bytes) != cudaSuccess || cudaMalloc(&c->held, copies * held_bytes) != cudaSuccess ||
       (q.beta_stencil && cudaMalloc(&c->cfield, c_bytes) != cudaSuccess) ||
       cudaMalloc((void **)&c->partials, (size_t)c->nblk_flat * 8 * sizeof(double)) != cudaSuccess ||
       cudaMalloc((void **)&c->diag_dev, 8 * sizeof(double)) != cudaSuccess ||
@@ -469,6 +496,10 @@ int lbm_create(int dim, int lattice, int nx, int ny, int nz, const lbm_params *p
     cudaGetLastError();
     lbm_destroy(c);
     return LBM_ENOMEM;
+  }
+  if (c->steps_1d) {
+    c->pop2 = (char *)c->pop + pop_bytes;
+    c->held2 = (char *)c->held + held_bytes;
   }
   *out = c;
   return LBM_OK;
@@ -550,12 +581,8 @@ static int enqueue_diag(lbm_ctx *c, double *dev_out) {
   return LBM_OK;
 }
 
-// One step: the launch, and the diagnostics every diag_every steps.
-static int one_step(lbm_ctx *c) {
-  StepArgs a = make_args(c, c->t);
-  CUDA_TRY(c, dispatch_step(c, a));
-  c->first_step = 0;
-  c->t++;
+// The diagnostics of a step that is due for them, enqueued after it.
+static int diag_if_due(lbm_ctx *c) {
   if (c->p.diag_every > 0 && (c->t % c->p.diag_every) == 0) {
     if (c->diag_pending) {
       int rc = check_diag(c, 1);
@@ -568,6 +595,15 @@ static int one_step(lbm_ctx *c) {
     c->diag_pending = 1;
   }
   return LBM_OK;
+}
+
+// One step: the launch, and the diagnostics every diag_every steps.
+static int one_step(lbm_ctx *c) {
+  StepArgs a = make_args(c, c->t);
+  CUDA_TRY(c, dispatch_step(c, a));
+  c->first_step = 0;
+  c->t++;
+  return diag_if_due(c);
 }
 
 static long long gcd_ll(long long a, long long b) { return b ? gcd_ll(b, a % b) : a; }
@@ -642,6 +678,44 @@ static int replay_period(lbm_ctx *c, int period) {
   return LBM_OK;
 }
 
+// Steps of a short FP64 1D lattice, several per launch: up to `left`, ending
+// where diagnostics are due (a whole period of the step arguments takes them
+// once, after its last step, as a replayed one does).
+static int steps_1d(lbm_ctx *c, long long left, long long *done) {
+  long long n = left;
+  if (c->p.diag_every > 0) {
+    const int period = graph_period(c);
+    if (period > 0 && c->t % period == 0 && left >= period) {
+      n = period;
+    } else {
+      const long long due = c->p.diag_every - c->t % c->p.diag_every;
+      n = left < due ? left : due;
+    }
+  }
+  *done = n;
+  while (n > 0) {
+    Ref1DArgs r;
+    r.a = make_args(c, c->t);
+    r.pop_out = (double *)c->pop2;
+    r.held_out = (double *)c->held2;
+    r.steps = (int)(n < c->steps_1d ? n : c->steps_1d);
+    while ((r.shift = r1_shift(c->n[0], r.steps, r.a.has_outlet)) < 0) r.steps--;
+    r.latch = 0;
+    for (int k = 0; k < r.steps; k++) {
+      if ((c->t + k) % c->p.n_gamma == 0 || (k == 0 && c->first_step)) r.latch |= 1u << k;
+      inlet_at(c->p, c->t + k, r.aIN[k], r.ugIN[k], r.ulIN[k]);
+    }
+    CUDA_TRY(c, launch_ref_steps_1d(r, c->stream));
+    c->launches++;
+    std::swap(c->pop, c->pop2);
+    std::swap(c->held, c->held2);
+    c->first_step = 0;
+    c->t += r.steps;
+    n -= r.steps;
+  }
+  return diag_if_due(c);
+}
+
 int lbm_step(lbm_ctx *c, int n) {
   if (!c || n < 0) return LBM_EINVAL;
   if (!c->initialised) return set_err(c, LBM_ESTATE, "lbm_step before lbm_init");
@@ -650,6 +724,13 @@ int lbm_step(lbm_ctx *c, int n) {
   if (rc) return rc;
   long long left = n;
   while (left > 0) {
+    if (c->pop2) {
+      long long k = 0;
+      rc = steps_1d(c, left, &k);
+      left -= k;
+      if (rc) return rc;
+      continue;
+    }
     const int period = graph_period(c);
     if (period > 0 && c->t % period == 0 && left >= period) {
       rc = replay_period(c, period);
@@ -770,8 +851,9 @@ const char *lbm_last_error(const lbm_ctx *c) { return c ? c->err : ""; }
 int lbm_destroy(lbm_ctx *c) {
   if (!c) return LBM_OK;
   if (c->stream || c->pop) cudaStreamSynchronize(c->stream);
-  if (c->pop) cudaFree(c->pop);
-  if (c->held) cudaFree(c->held);
+  // (of two copies in one allocation, whichever comes first)
+  if (c->pop) cudaFree(c->pop2 && c->pop2 < c->pop ? c->pop2 : c->pop);
+  if (c->held) cudaFree(c->held2 && c->held2 < c->held ? c->held2 : c->held);
   if (c->cfield) cudaFree(c->cfield);
   if (c->partials) cudaFree(c->partials);
   if (c->diag_dev) cudaFree(c->diag_dev);

@@ -12,6 +12,12 @@ struct lbm_ctx {
   long long N, plane;
   lbm_params p;
   void *pop = nullptr, *held = nullptr;
+  // short FP64 1D lattices (several steps per launch, lbm_ref_1d.cuh): the
+  // store and held fields the next launch writes, in one allocation with
+  // the ones it reads
+  void *pop2 = nullptr, *held2 = nullptr;
+  int steps_1d = 0;          // steps per launch (0: not such a lattice)
+  int sms = 1;               // SMs of the device
   void *cfield = nullptr;    // beta-stencil form: 2 x 2*D planes of c
   double *partials = nullptr, *diag_dev = nullptr;
   double *h_diag = nullptr;  // pinned, 8 doubles

@@ -457,6 +457,26 @@ __global__ void __launch_bounds__(256) k_step_ref(const StepArgs a) {
   else collide(std::true_type{});
 }
 
+// Several steps of a short 1D lattice in one launch (lbm_ref_1d.cuh)
+constexpr int R1_NODES = 16, R1_MAX_STEPS = 8;
+__host__ __device__ constexpr int r1_core(int steps) { return R1_NODES - 2 * (steps - 1); }
+// An outlet's rule needs its inward neighbour to the last step, so the last
+// node may not be the first core node of its warp (one more node of halo
+// would be needed on that side): the warps are moved by one node where it
+// would be.  -1: `steps` does not fit (cores of two nodes cannot be moved, an
+// inlet's neighbour would leave the halo on the other side).
+__host__ __device__ constexpr int r1_shift(int n, int steps, bool outlet) {
+  return !outlet || (n - 1) % r1_core(steps) != 0 ? 0 : (r1_core(steps) > 2 ? 1 : -1);
+}
+struct Ref1DArgs {
+  StepArgs a;  // pop, held: the store read; parity: of the first step
+  double *pop_out, *held_out;
+  int steps;
+  int shift;       // nodes by which the warps' first core node lies before node 0
+  unsigned latch;  // bit k: step k latches
+  double aIN[R1_MAX_STEPS], ugIN[R1_MAX_STEPS], ulIN[R1_MAX_STEPS];
+};
+
 // Initial equilibria (full values), Sec. 2 initial state: eps_g = p_k/cs2,
 // eps_l = 1, phi of Eq. (lbm-phi-l), alpha_l = 1 - alpha_g, c of Eq.
 // (velocitybeta); held S'' = 0, Lambda' = Lambda(alpha_g).

@@ -173,6 +173,34 @@ def test_fp64_reference_tiny_velocities_bitwise(lat, dims, scale):
             assert np.array_equal(got[k], ref[k]), (k, steps)
 
 
+@pytest.mark.parametrize("n", [2, 3, 7, 15, 16, 17, 64, 203, 305, 609, 1217, 2129, 2433, 4257])
+@pytest.mark.parametrize("case", ["walls", "periodic", "tube", "wall_outlet"])
+def test_fp64_1d_several_steps_per_launch_bitwise(n, case):
+    """Short FP64 1D lattices advance several steps per launch (lbm_ref_1d.cuh):
+    sizes about the blocks' cores and the counts of blocks at which the steps
+    per launch change, latches inside a launch, odd and even starts; the last
+    node in every place of its block (the outlet's neighbour).  Where a random
+    state is unstable beside an outlet, both become non-finite at the same
+    nodes."""
+    bc = {"walls": (WALL, WALL), "periodic": (PER, PER), "tube": (INLET, OUTLET), "wall_outlet": (WALL, OUTLET)}[case]
+    p = dict(R=30.0, omega_g=0.6, omega_l=1.2, omega_alpha=1.7, drag_model=int(case != "tube"), kappa_I=1e-3,
+             kappa_W=0.0 if case == "periodic" else 1e-3, psi_g=0.1, psi_l=0.2, g_hat=1e-6, g_axis=0, gamma=0.5,
+             n_gamma=1 if case == "tube" else 3, spalding_mode={"walls": 0, "wall_outlet": 1}.get(case, 2),
+             bc_lo=(bc[0], 0, 0), bc_hi=(bc[1], 0, 0), in_alpha=(0.05, 0.5), in_ug=(1e-3, 5e-3), in_ul=(0.0, 1e-3),
+             ramp_nt=20)
+    f = case_fields("D1Q3", (n,), seed=n)
+    o = oracle.Oracle("D1Q3", (n, 1, 1), p, threads=8)
+    o.init(**f)
+    s = lbm.Simulation("D1Q3", (n,), dict(p, precision="fp64", diag_every=0))
+    s.init(**f)
+    for steps in (1, 8, 3, 19):
+        o.step(steps)
+        s.step(steps)
+        got, ref = s.moments(), o.moments()
+        for k in ("alpha_g", "u_g", "u_l", "p_k", "S_g", "S_l"):
+            assert np.array_equal(got[k], np.asarray(ref[k]).reshape(got[k].shape), equal_nan=True), (k, s.t)
+
+
 @pytest.mark.parametrize("name", sorted(CASES))
 def test_parity_fp64dev(name):
     """The fast kernels' deviation arithmetic, in double.  Bar 1e-9: the
