@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "lbm_kernels.cuh"
+#include "lbm_launch_early.h"
 
 namespace lbm {
 
@@ -20,7 +21,7 @@ struct Launch {
   template <class K>
   static void go(K kern, const StepArgs &a, dim3 grid, dim3 block, size_t smem, cudaStream_t st) {
     if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<grid, block, smem, st>>>(a);
+    launch_early(kern, grid, block, smem, st, a);
   }
   template <bool BS, class OffT>
   static void step_form(int prec, const StepArgs &a, dim3 grid, dim3 block, size_t smem, cudaStream_t st) {
@@ -47,10 +48,10 @@ struct Launch {
   template <class OffT>
   static void batch_form(int prec, const StepArgs *args, const WorkItem *work, unsigned nwork, dim3 block,
                          int parity, int latch, cudaStream_t st) {
-    if (prec == 3) k_batch_step<L, double, double, OffT><<<nwork, block, 0, st>>>(args, work, parity, latch);
-    else if (prec == 1) k_batch_step<L, float, float, OffT><<<nwork, block, 0, st>>>(args, work, parity, latch);
-    else if (prec == 4) k_batch_step<L, MixAB, float, OffT><<<nwork, block, 0, st>>>(args, work, parity, latch);
-    else k_batch_step<L, __half, float, OffT><<<nwork, block, 0, st>>>(args, work, parity, latch);
+    if (prec == 3) launch_early(k_batch_step<L, double, double, OffT>, dim3(nwork), block, 0, st, args, work, parity, latch);
+    else if (prec == 1) launch_early(k_batch_step<L, float, float, OffT>, dim3(nwork), block, 0, st, args, work, parity, latch);
+    else if (prec == 4) launch_early(k_batch_step<L, MixAB, float, OffT>, dim3(nwork), block, 0, st, args, work, parity, latch);
+    else launch_early(k_batch_step<L, __half, float, OffT>, dim3(nwork), block, 0, st, args, work, parity, latch);
   }
   // off32: every instance has Q*plane < 2^32
   static cudaError_t batch_step(int prec, const StepArgs *args, const WorkItem *work, unsigned nwork, dim3 block,
