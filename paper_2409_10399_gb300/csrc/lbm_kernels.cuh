@@ -863,6 +863,12 @@ template <> struct StepBounds<Lattice<3>, MixAB> { static constexpr int threads 
 template <> struct StepBounds<Lattice<2>, MixAB> { static constexpr int threads = 128, blocks = 5; };
 template <> struct StepBounds<Lattice<1>, MixAB> { static constexpr int threads = 128, blocks = 4; };
 
+}  // namespace lbm
+
+#include "lbm_pairs.cuh"
+
+namespace lbm {
+
 // One node of the fused step (rows a1-a10).  `a` may live in kernel
 // parameter space (single lattice) or in global memory (batched instances);
 // parity and latch are the step's (t & 1, t % n_gamma == 0).  With
@@ -885,6 +891,10 @@ __device__ __forceinline__ void fused_step_node(const StepArgs &a, Geo &g, bool 
                                                 int latch, bool blk_xch, int gstride, R *xch,
                                                 const HaloStage &hs = HaloStage{nullptr, 0, 0, 0, {0, 0, 0}, 0}) {
   constexpr int D = L::D, Q = L::Q;
+  if constexpr (std::is_same<S, float>::value && !BS && D > 1) {
+    paired_step_node<L, OffT, IO>(a, g, active, tid, parity, latch, blk_xch, gstride, xch);
+    return;
+  } else {
   const int gax = a.g_axis;
   Pops<L, S, R, BS> f;
   Moments<L, R> m;
@@ -1320,6 +1330,7 @@ __device__ __forceinline__ void fused_step_node(const StepArgs &a, Geo &g, bool 
   };
   if (interior) collide_all(std::true_type{});
   else collide_all(std::false_type{});
+  }
 }
 
 // Programmatic dependent launch: a step's blocks may be scheduled while the
