@@ -20,7 +20,7 @@ struct lbm_ctx {
   int sms = 1;               // SMs of the device
   void *cfield = nullptr;    // beta-stencil form: 2 x 2*D planes of c
   double *partials = nullptr, *diag_dev = nullptr;
-  double *h_diag = nullptr;  // pinned, 8 doubles
+  double *h_diag = nullptr;  // pinned, 8 doubles, then sum and first bad index of an alpha_g check
   cudaEvent_t diag_ev = nullptr;
   int diag_pending = 0;
   unsigned nblk_flat = 0;
