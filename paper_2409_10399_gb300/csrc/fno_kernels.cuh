@@ -16,6 +16,10 @@ __device__ __forceinline__ float gelu(float z);
 
 // ---------------------------------------------------------------- elementwise
 
+// lets the next kernel of the stream (a product, which waits for this one's end
+// before it touches memory) be scheduled early
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // hardware tanh (PTX tanh.approx.f32, relative error ~2^-11): below the
 // 2^-9 of the BF16 activations it feeds
 __device__ __forceinline__ float tanh_fast(float x) {
@@ -37,6 +41,7 @@ __device__ __forceinline__ float gelu_grad(float z) {
 
 // dz = act ? dh * gelu'(z) : dh  (float and bf16 copies)
 __global__ void k_act_back(const float *dh, const float *z, float *dz, bf16 *dz16, long long n, int act) {
+  let_next_start();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float v = act ? dh[i] * gelu_grad(z[i]) : dh[i];
@@ -47,6 +52,7 @@ __global__ void k_act_back(const float *dh, const float *z, float *dz, bf16 *dz1
 // db[c] += sum_p dz[c][p]: blocks (chunk, c), each reducing its chunk of the
 // channel in a tree and adding it atomically
 __global__ void k_bias_grad(const float *dz, float *db, long long P) {
+  let_next_start();
   __shared__ float s[256];
   const int c = blockIdx.y;
   const long long chunk = (P + gridDim.x - 1) / gridDim.x, p0 = blockIdx.x * chunk;
@@ -134,6 +140,7 @@ __global__ void k_adam(float *p, const float *g, float *m, float *v, long long n
 }
 
 __global__ void k_to_bf16(const float *x, bf16 *y, long long n) {
+  let_next_start();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = __float2bfloat16(x[i]);
 }
@@ -157,6 +164,7 @@ __global__ void k_assemble_complex(const float *A, const float *B, bf16 *W, int 
 // gradient of the real 2C x 2C matrices back onto A_k, B_k:
 // dA = dW11 + dW22, dB = dW21 - dW12
 __global__ void k_fold_complex(const float *dW, float *dA, float *dB, int C, int K) {
+  let_next_start();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)K * C * C) return;
   const int k = (int)(i / ((long long)C * C));

@@ -253,6 +253,10 @@ __global__ void __launch_bounds__(UMMA_THREADS) k_umma(const __grid_constant__ U
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // launched while the kernel before it in the stream still runs: nothing above
+  // touches memory of others; below, that kernel has ended
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                  "r"(g.tmem_cols)
