@@ -48,11 +48,11 @@ FALLBACK_HBM_GBS = 6800.0
 STORE_BYTES = {"fp64": 8, "fp32": 4, "fp16dev": 2}
 HELD_BYTES = {"fp64": 8, "fp32": 4, "fp16dev": 4}
 Q_OF = {"D1Q3": 3, "D2Q9": 9, "D3Q19": 19}
-KERNEL_SRC = os.path.join(ROOT, "paper_2409_10399_gb300", "csrc", "lbm_kernels.cuh")
+KERNEL_SRC = [os.path.join(ROOT, "paper_2409_10399_gb300", "csrc", f) for f in ("lbm_kernels.cuh", "lbm_pairs.cuh")]
 # DRAM bytes (read + write) per launch of the box2d FP32 step kernel from one
 # ncu capture, valid only for the kernel source it was taken on (the SHA-256
-# prefix of lbm_kernels.cuh); otherwise the bench reports traffic null.
-NCU_TRAFFIC = {"kernel_source_sha16": "b364f640c0f2b1e3", "bytes_per_launch": 408036352.0}
+# prefix of lbm_kernels.cuh and lbm_pairs.cuh); otherwise the bench reports traffic null.
+NCU_TRAFFIC = {"kernel_source_sha16": "5c0e59b909a4ec8d", "bytes_per_launch": 419645696.0}
 
 
 def bytes_per_node(lattice, prec):
@@ -79,7 +79,7 @@ def measured_peak():
 
 
 def kernel_hash():
-    return hashlib.sha256(open(KERNEL_SRC, "rb").read()).hexdigest()[:16]
+    return hashlib.sha256(b"".join(open(f, "rb").read() for f in KERNEL_SRC)).hexdigest()[:16]
 
 
 def ncu_traffic():
