@@ -46,6 +46,9 @@ from . import params as lparams
 # (column1d 512, box2d at 512 x 256, column3d at 64 x 64 x 128), divided by the
 # nodes.  The dfma come mostly from the IEEE division and square root
 # sequences: the reference evaluates the paper's divisions literally.
+# (operations of the step with IEEE division sequences, the scale in which the
+# reference path is reported; it executes fewer since its divisions by the lattice
+# constants take two, so the fraction can come near 1 and above)
 FP64_OPS_PER_NODE = {"D1Q3": 710, "D2Q9": 1956, "D3Q19": 4219}
 B6 = {("D2Q9", "fp32"): 444, ("D2Q9", "fp16dev"): 228, ("D2Q9", "fp64"): 888,
       ("D3Q19", "fp32"): 924, ("D3Q19", "fp16dev"): 468, ("D3Q19", "fp64"): 1848,
