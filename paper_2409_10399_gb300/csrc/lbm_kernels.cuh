@@ -1344,15 +1344,22 @@ __device__ __forceinline__ void fused_step_node(const StepArgs &a, Geo &g, bool 
 }
 
 // Programmatic dependent launch: a step's blocks may be scheduled while the
-// last ones of the kernel before it in the stream still run (they are let go
-// at once), and wait here for its end and its stores before their first
-// access to memory.  It hides the launch and the empty tail of a step: 2 us
-// of each (2D box, FP16AB store, 71.4 -> 68.8 us; 256 x 1024 nodes FP32 16.5
-// -> 14.6).  Not in the FP64 kernels: waiting blocks slowed the short 1D ones by
-// two thirds (512 nodes 6.1 -> 10.2 us a step).
+// kernel before it in the stream still runs, and wait here for its end and its
+// stores before their first access to memory.  It hides the launch and the
+// empty tail of a step.  A step lets the next one go only after its own wait:
+// let go before it, the blocks of several steps to come gather on the SMs when
+// a step has fewer blocks than fit at once, take the places of the step that
+// is due and crowd its blocks onto few SMs.
+// Measured (us a step; no overlap / let go before the wait / after it): D1Q3
+// of 20,000 nodes FP32 2.71 / 3.16 / 2.08, of 8,192 in FP64DEV 12.3 / 30.3 / 11.3;
+// D2Q9 of 100 x 200 FP32 6.17 / 6.39 / 3.94, of 256 x 1024 16.7 / 14.60 / 14.71, of
+// 512 x 2048 79.5 / 76.3 / 76.4, FP16AB 71.0 / 68.1 / 68.2; D3Q19 of 32^3 FP16
+// 8.3 / 7.7 / 5.7, of 128^3 195.6 / 193.0 / 193.1.  After the loads instead, the
+// 512 x 2048 box takes 82.5; before or after by the size of the grid, the
+// branch costs the large ones as much as it gives (128^3 FP16 195.4).
 __device__ __forceinline__ void wait_previous() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <class L, class S, class R, bool BS, class OffT, bool IO = true>

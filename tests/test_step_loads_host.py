@@ -65,3 +65,10 @@ def test_the_batch_reads_only_its_constant_tables_early():
     wait = body.index("wait_previous")
     assert [m.group(0) for m in READ_ONLY.finditer(body)] == ["__restrict__", "__restrict__", "__ldg"]
     assert "a.pop" not in body[:wait] and not READ_ONLY.search(body[wait:])
+
+
+def test_a_step_lets_the_next_go_after_its_own_wait():
+    """Let go before the wait, the blocks of several steps to come would hold
+    the SMs that a step of few blocks needs."""
+    (body,) = _bodies(_source("lbm_kernels.cuh"), "wait_previous")
+    assert 0 < body.index("griddepcontrol.wait") < body.index("griddepcontrol.launch_dependents")
