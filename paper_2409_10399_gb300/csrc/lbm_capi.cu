@@ -729,9 +729,14 @@ static int replay_period(lbm_ctx *c, int period) {
   return LBM_OK;
 }
 
-// Steps of a short FP64 1D lattice, several per launch: up to `left`, ending
-// where diagnostics are due (a whole period of the step arguments takes them
-// once, after its last step, as a replayed one does).
+// Steps of a short FP64 1D lattice, several per launch: up to `left` (what
+// remains of the caller's), ending where diagnostics are due (a whole period
+// of the step arguments takes them once, after its last step, as a replayed
+// one does).  A launch moves the state from one copy of the store to the
+// other, and every lbm_step takes an even number of them (a last step may be
+// taken in place): the state is back in the first copy when the call returns,
+// so that a caller may capture a call and replay it, plain calls in between.
+// It costs a launch in every second call, 5 us.
 static int steps_1d(lbm_ctx *c, long long left, long long *done) {
   long long n = left;
   if (c->p.diag_every > 0) {
@@ -744,13 +749,20 @@ static int steps_1d(lbm_ctx *c, long long left, long long *done) {
     }
   }
   *done = n;
+  const bool last = n == left;
   while (n > 0) {
     Ref1DArgs r;
     r.a = make_args(c, c->t);
-    r.pop_out = (double *)c->pop2;
-    r.held_out = (double *)c->held2;
-    r.steps = (int)(n < c->steps_1d ? n : c->steps_1d);
-    while ((r.shift = r1_shift(c->n[0], r.steps, r.a.has_outlet)) < 0) r.steps--;
+    auto fit = [&](long long want) {
+      r.steps = (int)(want < c->steps_1d ? want : c->steps_1d);
+      while ((r.shift = r1_shift(c->n[0], r.steps, r.a.has_outlet)) < 0) r.steps--;
+    };
+    fit(n);
+    const bool odd = last && r.steps == n && c->pop < c->pop2;  // the last launch would end in the second copy
+    if (odd && n > 1) fit((n + 1) / 2);
+    const bool in_place = odd && n == 1;
+    r.pop_out = (double *)(in_place ? c->pop : c->pop2);
+    r.held_out = (double *)(in_place ? c->held : c->held2);
     r.latch = 0;
     for (int k = 0; k < r.steps; k++) {
       if ((c->t + k) % c->p.n_gamma == 0 || (k == 0 && c->first_step)) r.latch |= 1u << k;
@@ -758,8 +770,10 @@ static int steps_1d(lbm_ctx *c, long long left, long long *done) {
     }
     CUDA_TRY(c, launch_ref_steps_1d(r, c->stream));
     c->launches++;
-    std::swap(c->pop, c->pop2);
-    std::swap(c->held, c->held2);
+    if (!in_place) {
+      std::swap(c->pop, c->pop2);
+      std::swap(c->held, c->held2);
+    }
     c->first_step = 0;
     c->t += r.steps;
     n -= r.steps;
