@@ -393,7 +393,13 @@ __global__ void __launch_bounds__(UMMA_THREADS) k_umma(const __grid_constant__ U
       const bool has = iters1(kbeg, kend) + nk2 > 0;
       const int n = n0 + row;
       const bool n_in = n < g.N;
-      const float bz = bias_z ? g.bias[zb] : 0.0f;
+      // (the bias may be read as read-only data although the block lives while
+      // the kernel before it ends: parameters are written by the optimiser's
+      // kernel and by copies alone, and kernels launched in full order follow
+      // those before the next product; by ordinary loads, which the epilogue's
+      // stores hold back, 64 x 262144 x 64 with FP32 output takes 24.9 us
+      // instead of 23.9, bias or not)
+      const float bz = bias_z ? __ldg(g.bias + zb) : 0.0f;
       // row m of the output at element offset mrow(m) + n
       const long long cb = (long long)zb * g.sC + n;
       const float *old = oldc + b * (SM::OLD_TILE / 4) + row;  // nacc tiles of NT x 128
@@ -432,7 +438,7 @@ __global__ void __launch_bounds__(UMMA_THREADS) k_umma(const __grid_constant__ U
         }
         if (bias_r) {
 #pragma unroll
-          for (int jj = 0; jj < 16; jj++) o[jj] += mc + jj < g.M ? g.bias[mc + jj] : 0.0f;
+          for (int jj = 0; jj < 16; jj++) o[jj] += mc + jj < g.M ? __ldg(g.bias + mc + jj) : 0.0f;
         } else if (bias_z) {
 #pragma unroll
           for (int jj = 0; jj < 16; jj++) o[jj] += bz;
