@@ -30,12 +30,13 @@ namespace lbm {
 // 12.6, 200 nodes with inlet and outlet 7.7 against 21.0; about 5.3 us a step
 // plus 5 us a launch while an SM holds one block, 8.8 us with two.
 
-// |x| = sqrt(x x): exact in radix 2 unless x x leaves the normal range (S.
+// |x| = sqrt(x x): exact in radix 2 unless x x leaves the normal range (below
+// 2^-300 and for all finite x from 2^500 on the formula as it stands is taken; S.
 // Boldo, "Stupid is as stupid does: taking the square root of the square of
 // a floating-point number", 2015)
 __device__ __forceinline__ double r1_abs(double x) {
   const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
-  if (ref_small(x) || h - ((1023u + 500u) << 20) < (500u << 20)) return sqrt(x * x);
+  if (ref_small(x) || h - ((1023u + 500u) << 20) < (524u << 20)) return sqrt(x * x);
   return fabs(x);
 }
 // first + x/cs2 + quad and first - x/cs2 + quad, x = v.u of the +1 direction
