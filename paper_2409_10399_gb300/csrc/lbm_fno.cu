@@ -287,7 +287,8 @@ static cudaError_t launch_umma(fno::UmmaArgs &a, int nk, bool want_c, bool want_
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = early ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, a);
+  cudaLaunchKernelEx(&cfg, kern, a);
+  return cudaGetLastError();  // its status, and none left for a later call
 }
 
 template <bool AK, bool BKM>
