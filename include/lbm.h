@@ -129,8 +129,9 @@ void lbm_default_params(lbm_params *p);
  * (ny = nz = 1 for D1Q3, nz = 1 for D2Q9).  Validates rates, sizes and
  * boundary codes (LBM_EINVAL), allocates 6*Q*N populations (4*Q*N plus
  * 4*D*N values of c with beta_stencil) plus three held fields (S''_g,
- * S''_l, Lambda') and small scratch on the current CUDA device
- * (LBM_ENOMEM).  *out is NULL on failure. */
+ * S''_l, Lambda') and small scratch on the current CUDA device, populations
+ * and held fields twice for the short LBM_FP64 D1Q3 lattices named at
+ * lbm_set_graph (LBM_ENOMEM).  *out is NULL on failure. */
 int lbm_create(int dim, int lattice, int nx, int ny, int nz, const lbm_params *p, lbm_ctx **out);
 
 /* Set every scheme to its equilibrium from macroscopic fields and reset t = 0:
@@ -187,7 +188,11 @@ int lbm_get_diag(lbm_ctx *c, double out[8]);
  * taken once, after its last step (the period is a multiple of diag_every),
  * so a non-finite state or a drift is reported at most one period after it
  * arises.  enable = 0 launches every step.  lbm_init and
- * lbm_set_tile drop the captured graph.  Not in the paper. */
+ * lbm_set_tile drop the captured graph.  Short LBM_FP64 D1Q3 lattices (up to
+ * some 4,000 nodes: two blocks of 14 nodes on every SM) use no graph: they
+ * advance up to eight steps per launch either way, ending a launch where
+ * diagnostics are due; enable still chooses between diagnostics once per
+ * period and at every due step.  Not in the paper. */
 int lbm_set_graph(lbm_ctx *c, int enable);
 
 /* Use `cuda_stream` (a cudaStream_t of the current device, e.g. the value of
@@ -200,7 +205,9 @@ int lbm_set_stream(lbm_ctx *c, void *cuda_stream);
  * or 256 (the other lattices and precisions).  The default is chosen at
  * lbm_create; an autotuner may try others.  With an inlet or outlet face the
  * tile along g_axis must be >= 2 (LBM_EINVAL otherwise).  Takes effect at the
- * next lbm_step; results do not depend on the tile. */
+ * next lbm_step; results do not depend on the tile.  It has no effect on the
+ * short LBM_FP64 D1Q3 lattices named at lbm_set_graph, whose kernel has a
+ * block of its own. */
 int lbm_set_tile(lbm_ctx *c, int tx, int ty, int tz);
 
 /* Current tile (tile[0..2]) of the fused step kernel. */

@@ -3,7 +3,8 @@
 Times each candidate thread-block tile for a few steps on the caller's own
 state (CUDA events on the current stream), keeps the fastest, and caches the
 choice per (GPU, lattice, precision, problem size class) in a JSON file next
-to the built library.  Results never depend on the tile, so tuning is safe on
+to the built library.  The tile has no effect on short FP64 1D lattices (a few
+thousand nodes; lbm_set_tile in lbm.h).  Results never depend on the tile, so tuning is safe on
 a live state; the steps it takes advance the state.
 """
 import json
@@ -49,13 +50,21 @@ def _size_class(nodes):
     return "2^%d" % max(0, int(nodes).bit_length() - 1)
 
 
+def _size_key(lattice_d, precision, nodes):
+    """The sizes that share a tuned tile.  Short FP64 1D lattices advance
+    several steps per launch with a block of their own, whatever the tile, so
+    what is timed on them says nothing about a longer one: every length is
+    tuned by itself there."""
+    return "n=%d" % nodes if lattice_d == 1 and precision == "fp64" else _size_class(nodes)
+
+
 def tune(obj, lattice_d, precision, nodes, kind, steps=40, use_cache=True):
     """Choose a tile for `obj` (a Simulation or a Batch: set_tile, step).
     Returns (tile, {tile: seconds per step})."""
     import torch
     from . import tile_limit
     maxthr = tile_limit(lattice_d, precision)
-    key = "|".join([_gpu_name(), "D%d" % lattice_d, precision, kind, _size_class(nodes)])
+    key = "|".join([_gpu_name(), "D%d" % lattice_d, precision, kind, _size_key(lattice_d, precision, nodes)])
     cache = _load() if use_cache else {}
     if key in cache:
         tile = tuple(cache[key]["tile"])

@@ -83,3 +83,25 @@ def test_tune_keeps_the_fastest_and_caches(monkeypatch, tmp_path):
     autotune.tune(obj, 2, "fp32", 1 << 22, "single", steps=10)
     assert obj.steps > steps
     assert autotune._size_class(1 << 20) == autotune._size_class((1 << 21) - 1) != autotune._size_class(1 << 21)
+
+
+def test_1d_fp64_lengths_are_tuned_one_by_one(monkeypatch, tmp_path):
+    """A short FP64 1D lattice ignores the tile (several steps per launch), so
+    what was timed on it is not taken for a longer one of its size class."""
+    monkeypatch.setattr(autotune, "CACHE", str(tmp_path / "tiles.json"))
+    tiles = autotune.CANDIDATES[(1, 256)]
+    short = _Fake({t: 1e-5 for t in tiles}, reject=())
+    short.cost[tiles[0]] = 0.9e-5  # noise
+    _fake_cuda(monkeypatch, short)
+    autotune.tune(short, 1, "fp64", 4200, "single", steps=10)
+    longer = _Fake({t: 1e-5 * (1 + i) for i, t in enumerate(reversed(tiles))}, reject=())
+    _fake_cuda(monkeypatch, longer)
+    tile, times = autotune.tune(longer, 1, "fp64", 5000, "single", steps=10)
+    assert longer.steps > 0 and tile == tiles[-1] and set(times) == set(tiles)
+    # other lattices of a size class still share their choice
+    one = _Fake({t: 1e-5 for t in autotune.CANDIDATES[(1, 128)]}, reject=())
+    _fake_cuda(monkeypatch, one)
+    autotune.tune(one, 1, "fp32", 4200, "single", steps=10)
+    steps = one.steps
+    autotune.tune(one, 1, "fp32", 5000, "single", steps=10)
+    assert one.steps == steps
