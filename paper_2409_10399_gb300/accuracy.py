@@ -124,10 +124,12 @@ def main():
     todo = []
     if args.study == "fp64_launches":
         # two launches of the FP64 reference step on each workload recipe at
-        # a size one capture can hold (the FP64 operation counts of the
-        # reference kernels are taken with ncu on these launches)
-        todo.append(lambda: [throughput(n, "fp64", steps=2, dims=d, warm=0) for n, d in
-                             (("column1d", (512, 1, 1)), ("box2d", (512, 256, 1)), ("column3d", (64, 64, 128)))])
+        # a size one capture can hold, seven steps each of the 1D column (the
+        # FP64 operation counts of the reference kernels are taken with ncu on
+        # these launches)
+        todo.append(lambda: [throughput(n, "fp64", steps=k, dims=d, warm=0) for n, d, k in
+                             (("column1d", (512, 1, 1), 14), ("box2d", (512, 256, 1), 2),
+                              ("column3d", (64, 64, 128), 2))])
     if args.study == "column3d_small":
         # D3Q19 at 128 x 128 x 256 (2 GB of store traffic per step): the
         # profiling case of the 3D kernels

@@ -91,3 +91,17 @@ def test_clock_sampler_parses_nvidia_smi_lines():
     assert c == {"sm_mhz": 2050.0, "sm_max_mhz": 2070.0, "reasons": ["hw_slowdown", "sw_power_cap"], "samples": 3}
     empty = bench.ClockSampler(0)
     assert empty.stop() is None
+
+
+def test_reported_fp64_fractions_count_what_is_executed(monkeypatch):
+    """The forms' FP64 roofline at measured rates (573, 300 and 82 MLUPS against
+    1.10 TFLOP/s): a fraction of the peak, not of what an older step executed."""
+    rates = {"box2d": 573.0, "column3d": 300.0, "column1d": 82.0}
+    for name, v in rates.items():
+        monkeypatch.setattr(forms, name, lambda stream, quick, v=v: {"forms": {"fp64": {"MLUPS": v}}})
+    monkeypatch.setattr(forms, "fp64_peak", lambda: 1.10e12)
+    out = forms.all_forms(None, only=set(rates), quick=True)
+    for name, lat in (("box2d", "D2Q9"), ("column3d", "D3Q19"), ("column1d", "D1Q3")):
+        r = out[name]["forms"]["fp64"]["roofline"]
+        assert r["ops_per_node"] == forms.FP64_OPS_EXECUTED[lat]
+        assert 0.0 < r["frac"] < 1.0 and r["frac"] == pytest.approx(r["ops_per_node"] * rates[name] * 1e6 / 1.10e12)
