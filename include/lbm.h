@@ -150,8 +150,7 @@ int lbm_init(lbm_ctx *c, const double *alpha_g, const double *u_g, const double 
  * diag_every > 0 it also checks the diagnostics it has already received
  * (LBM_ENAN, LBM_EDRIFT).  LBM_ESTATE before lbm_init or after a sticky
  * error.
- * A call leaves the lattice's state in the memory where it found it.  So a
- * caller may capture, with graph replay off (lbm_set_graph) and diag_every =
+ * A caller may capture, with graph replay off (lbm_set_graph) and diag_every =
  * 0, calls that cover whole periods of the step arguments (an even number of
  * steps, a multiple of n_gamma, no inlet ramp) into a graph of its own and
  * replay it from the same phase of the period, between other calls too. */

@@ -775,10 +775,11 @@ static int replay_period(lbm_ctx *c, int period) {
 // remains of the caller's), ending where diagnostics are due (a whole period
 // of the step arguments takes them once, after its last step, as a replayed
 // one does).  A launch moves the state from one copy of the store to the
-// other, and every lbm_step takes an even number of them (a last step may be
-// taken in place): the state is back in the first copy when the call returns,
-// so that a caller may capture a call and replay it, plain calls in between.
-// It costs a launch in every second call, 5 us.
+// other.  From the first call on that a caller captures, every lbm_step takes
+// an even number of them (a last single step is k_step_ref's, in place): the
+// state is back in the copy that the capture read when the call returns, so that the
+// captured call can be replayed, plain calls in between.  That costs a launch,
+// 5 us, in every second call, which lattices that are never captured do not pay.
 static int steps_1d(lbm_ctx *c, long long left, long long *done) {
   long long n = left;
   if (c->p.diag_every > 0) {
@@ -792,6 +793,11 @@ static int steps_1d(lbm_ctx *c, long long left, long long *done) {
   }
   *done = n;
   const bool last = n == left;
+  if (!c->home) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
+    else if (st == cudaStreamCaptureStatusActive) c->home = c->pop;
+  }
   while (n > 0) {
     Ref1DArgs r;
     r.a = make_args(c, c->t);
@@ -800,11 +806,16 @@ static int steps_1d(lbm_ctx *c, long long left, long long *done) {
       while ((r.shift = r1_shift(c->n[0], r.steps, r.a.has_outlet)) < 0) r.steps--;
     };
     fit(n);
-    const bool odd = last && r.steps == n && c->pop < c->pop2;  // the last launch would end in the second copy
-    if (odd && n > 1) fit((n + 1) / 2);
-    const bool in_place = odd && n == 1;
-    r.pop_out = (double *)(in_place ? c->pop : c->pop2);
-    r.held_out = (double *)(in_place ? c->held : c->held2);
+    const bool odd = last && r.steps == n && c->pop == c->home;  // the last launch would end in the other copy
+    if (odd && n == 1) {
+      CUDA_TRY(c, dispatch_step(c, r.a));
+      c->first_step = 0;
+      c->t++;
+      break;
+    }
+    if (odd) fit((n + 1) / 2);
+    r.pop_out = (double *)c->pop2;
+    r.held_out = (double *)c->held2;
     r.latch = 0;
     for (int k = 0; k < r.steps; k++) {
       if ((c->t + k) % c->p.n_gamma == 0 || (k == 0 && c->first_step)) r.latch |= 1u << k;
@@ -812,10 +823,8 @@ static int steps_1d(lbm_ctx *c, long long left, long long *done) {
     }
     CUDA_TRY(c, launch_ref_steps_1d(r, c->stream));
     c->launches++;
-    if (!in_place) {
-      std::swap(c->pop, c->pop2);
-      std::swap(c->held, c->held2);
-    }
+    std::swap(c->pop, c->pop2);
+    std::swap(c->held, c->held2);
     c->first_step = 0;
     c->t += r.steps;
     n -= r.steps;

@@ -16,6 +16,7 @@ struct lbm_ctx {
   // store and held fields the next launch writes, in one allocation with
   // the ones it reads
   void *pop2 = nullptr, *held2 = nullptr;
+  void *home = nullptr;      // pop where a caller first captured a step (every call ends there)
   int steps_1d = 0;          // steps per launch (0: not such a lattice)
   int sms = 1;               // SMs of the device
   void *cfield = nullptr;    // beta-stencil form: 2 x 2*D planes of c

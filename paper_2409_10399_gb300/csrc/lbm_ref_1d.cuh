@@ -20,9 +20,7 @@ namespace lbm {
 //    nodes also holds the steps - 1 nodes beyond its core on either side
 //    (each step makes one more of them stale) and stores its core only.  The
 //    launch reads one store and writes another (pop_out, held_out), so no
-//    block reads what another writes.  A launch of one step has no such nodes
-//    and may write the store it reads: its slots are its node's own (the rule
-//    of the in-place step), each read and written by one lane.
+//    block reads what another writes.
 // The expressions and their order are those of k_step_ref, and so are the
 // results, bit for bit.
 // Measured (us per step; against k_step_ref, a thread per node and a launch
@@ -61,7 +59,7 @@ __global__ void __launch_bounds__(8 * R1_NODES) k_steps_ref_1d(const __grid_cons
   const bool per = a.bc_lo[0] == BC_PERIODIC;
   const int xl = (int)blockIdx.x * core - r.shift - (H - 1) + i;  // on the unrolled line
   const int x = per ? ((xl % N) + N) % N : xl;
-  const bool in = x >= 0 && x < N && (H > 1 || (xl >= 0 && xl < N)) && !isX;
+  const bool in = x >= 0 && x < N && !isX;
   const bool lo = !per && x == 0, hi = !per && x == N - 1;
   const bool mine = i >= H - 1 && i < H - 1 + core && xl >= 0 && xl < N && !isX;
   // does the block hold a face node with a rule (block-uniform)?
@@ -211,7 +209,6 @@ __global__ void __launch_bounds__(8 * R1_NODES) k_steps_ref_1d(const __grid_cons
       f2 = lo ? o1 : move[p][1][tl];
     }
   }
-  __syncwarp();  // (in place) a node's lanes have all read its held values
   if (!mine) return;
   // the last step's store: slot (x, opp q) on even steps and behind a face,
   // (x + v_q, q) on odd ones

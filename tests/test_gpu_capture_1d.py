@@ -1,8 +1,9 @@
 """A caller's own capture of lbm_step on a short FP64 1D lattice (several steps
-per launch, two copies of the store): every call leaves the state where it
-found it, so a captured call can be replayed, between plain calls too, whether
-the steps of a call divide by the steps of a launch or not.  Against the same
-steps taken by plain calls, bit for bit."""
+per launch, two copies of the store): once captured, a lattice's calls leave the
+state where the capture read it, so a captured call can be replayed, between
+plain calls too, whether the steps of a call divide by the steps of a launch or
+not, and from whichever copy the capture started.  Against the same steps taken
+by plain calls, bit for bit."""
 import numpy as np
 import pytest
 
@@ -29,14 +30,20 @@ def _sim(n, case, n_gamma, stream=None):
 
 @pytest.mark.parametrize("n, case", [(64, "walls"), (300, "periodic"), (201, "tube"), (512, "walls"), (3000, "walls"),
                                      (4257, "periodic")])
+@pytest.mark.parametrize("before", [False, True])
 @pytest.mark.parametrize("calls", [(2,), (1, 1), (6,), (7, 1), (10,), (200,), (3, 15)])
-def test_captured_calls_replay(n, case, calls):
+def test_captured_calls_replay(n, case, calls, before):
     import torch
     period = sum(calls)  # even, and a whole number of latches
     n_gamma = period if period in (2, 10, 200) else 2
     stream = torch.cuda.Stream()
     a, b = _sim(n, case, n_gamma, stream), _sim(n, case, n_gamma)
     a.step(period)
+    if before:  # other numbers of launches before the capture
+        for _ in range(period):
+            a.step(1)
+        a.step(period)
+        a.step(period)
     stream.synchronize()
     g = torch.cuda.CUDAGraph()
     with torch.cuda.graph(g, stream=stream):
@@ -49,7 +56,7 @@ def test_captured_calls_replay(n, case, calls):
         for _ in range(2):
             g.replay()
     stream.synchronize()
-    b.step(period + 3 * period + 2 * period + 2 * period)
+    b.step((1 + 3 * before) * period + 3 * period + 2 * period + 2 * period)
     ma, mb = a.moments(), b.moments()
     for k in mb:
         assert np.isfinite(mb[k]).all(), k
