@@ -854,14 +854,16 @@ __device__ __forceinline__ R feqS_dev(int q, R alpha, const R u[3], R uu, R r) {
 constexpr int XCH = 14;
 
 // Launch bounds of the fused step.  D2Q9 in float/half: at most 128 threads
-// and 5 resident blocks per SM, which caps registers at 102 (no spills) and
-// gives 20 warps per SM -- the kernel is memory-latency bound, and this
-// occupancy measured 11.8 GLUPS on the 512 x 2048 box against 11.1 GLUPS at
-// 104 registers / 16 warps (128 x 4, 128 x 6 and 256 x 3 were slower too).
-// D3Q19 in float/half: 128 threads, 3 blocks per SM (168 registers, a few
-// spills, 12 warps per SM); on the 256 x 256 x 512 column this measured
-// 6.11 / 4.85 GLUPS (FP16 / FP32 store) against 5.44 / 4.67 GLUPS with
-// 256 x 1 (249 registers, 8 warps).  The double forms keep 256 threads.
+// and 5 resident blocks per SM, which caps registers at 102 and gives 20
+// warps per SM -- the kernel is memory-latency bound; an early scalar FP32
+// form measured 11.8 GLUPS on the 512 x 2048 box against 11.1 GLUPS at 104
+// registers / 16 warps (128 x 4, 128 x 6 and 256 x 3 were slower too).
+// D3Q19 in float: 128 threads, 3 blocks per SM (168 registers, a few spills, 12
+// warps per SM), 4.85 GLUPS of the scalar form on the 256 x 256 x 512 column
+// against 4.67 with 256 x 1 (249 registers, 8 warps); in half 5 blocks (96
+// registers), 10.9 GLUPS against 8.7 and 9.1 with 3 and 6.  The paired FP32
+// form (lbm_pairs.cuh) was measured at one block more and one less too, 2D and
+// 3D, and keeps these bounds.  The double forms keep 256 threads.
 template <class L, class S> struct StepBounds { static constexpr int threads = 256, blocks = 1; };
 template <> struct StepBounds<Lattice<3>, float> { static constexpr int threads = 128, blocks = 3; };
 template <> struct StepBounds<Lattice<3>, __half> { static constexpr int threads = 128, blocks = 5; };
@@ -879,7 +881,9 @@ template <> struct StepBounds<Lattice<1>, MixAB> { static constexpr int threads 
 
 namespace lbm {
 
-// One node of the fused step (rows a1-a10).  `a` may live in kernel
+// One node of the fused step (rows a1-a10): this body for the half and FP16AB
+// stores, FP64DEV, the beta-stencil form and D1Q3; D2Q9 and D3Q19 in FP32 with six
+// schemes take paired_step_node (lbm_pairs.cuh), the same method.  `a` may live in kernel
 // parameter space (single lattice) or in global memory (batched instances);
 // parity and latch are the step's (t & 1, t % n_gamma == 0).  With
 // blk_xch the block exchanges the edge rows' values for the inlet/outlet
@@ -1202,8 +1206,7 @@ __device__ __forceinline__ void fused_step_node(const StepArgs &a, Geo &g, bool 
   // over 10,000 steps).
   // The rest direction's four populations wait in shared memory through the
   // pair loop (float arithmetic: four live registers fewer, so fewer spills
-  // inside the loop; box2d FP32 99 -> 80 us, FP16AB 77 -> 72 us), a slot per
-  // thread.
+  // inside the loop; 2D box FP16AB 77 -> 72 us), a slot per thread.
   constexpr bool STASH = std::is_same<R, float>::value;
   constexpr int NST = StepBounds<L, S>::threads;
   __shared__ R rest_stash[STASH ? 4 * NST : 1];

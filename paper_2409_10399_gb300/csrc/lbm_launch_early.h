@@ -5,7 +5,8 @@
 namespace lbm {
 
 // Launch whose blocks may be scheduled before the end of the kernel before it
-// (wait_previous in the kernel)
+// (wait_previous in the kernel).  As after <<<>>>, a refused launch is what the
+// caller's next cudaGetLastError returns.
 template <class K, class... A>
 static void launch_early(K kern, dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};

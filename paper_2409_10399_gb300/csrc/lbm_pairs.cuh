@@ -4,14 +4,12 @@
 // order.  Not for the stores with half planes: their rounding feeds back on
 // itself, so that any other rounding of the arithmetic leaves the fields as far
 // from the scalar form's as both are from the exact ones; nor for D1Q3.
-// Measured (us per step, scalar -> paired):
-// 2D box of 512 x 2048 with its inlet 80.4 -> 79.8 and 256 x 1024 18.4 -> 14.6
-// (launches overlapped in the second figures), 3D column of 256 x 256 x 128
-// 1,648 -> 1,386, 150 x 122 x 250 994 -> 821, 48 ragged 2D columns 1,598 ->
-// 1,423.  2D: instructions 49.2 -> 36.0 M
-// per launch, and the step waits on memory (6.2 long-scoreboard stalls per
-// issue); more warps would help, but the registers of five blocks are all taken
-// (StepBounds).
+// Measured (us per step; scalar and launched in order -> paired and overlapped):
+// 2D box of 512 x 2048 with its inlet 80.3 -> 79.8, 256 x 1024 16.8 -> 14.5, 3D column
+// of 256 x 256 x 128 1,647 -> 1,423, of 150 x 122 x 250 996 -> 839, 48 ragged 2D
+// columns 1,559 -> 1,427.  2D: instructions 49.2 -> 36.5 M per launch, and
+// the step waits on memory (6.2 long-scoreboard stalls per issue); more warps
+// would help, but the registers of five blocks are all taken (StepBounds).
 #pragma once
 
 namespace lbm {
@@ -407,7 +405,8 @@ __device__ __forceinline__ void paired_step_node(const StepArgs &a, Geo &g, bool
   // Collisions: the moving directions in pairs (q, opp q), q the one whose first
   // component is +1, the rest direction last, its non-equilibrium part the
   // remainder of theirs (fused_step_node says why, and why the hi + lo forms).
-  // The rest direction's four populations wait in shared memory meanwhile.
+  // The rest direction's four populations wait in shared memory meanwhile: four live
+  // registers fewer, so fewer spills (the scalar form's 2D box 99 -> 80 us).
   constexpr int NST = StepBounds<L, float>::threads;
   __shared__ float rest_stash[4 * NST];
   volatile R *const stash = rest_stash + threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
@@ -447,9 +446,11 @@ __device__ __forceinline__ void paired_step_node(const StepArgs &a, Geo &g, bool
       const Two F = O::mul(w, eLq), Hf = O::mul(aw, vG);
       // f_alpha: alpha^B = a + c (c the renormalisation, Spalding mode 2)
       const Two Xa = O::mul(w, m.da);
-      // (the two groupings of the same sum: with an inlet the shorter one's code
-      // spills where it hurts, 2D box 85.7 us a step against 79.8; without, 256 x
-      // 1024 14.6 against 15.0)
+      // (Two groupings of the same sum, by the lattice and the rules compiled in,
+      // not by size.  D2Q9 is held to 96 registers for its five blocks: with an
+      // inlet the shorter grouping's code spills where it hurts, 2D box 85.7 us a
+      // step against 79.8; without, 256 x 1024 14.6 against 15.0.  To be measured
+      // again when the launch bounds, the face rules or the compiler change.)
       Two Xal;
       if (IO && Q == 9) {
         Xal = O::add(O::add(O::fms(w, m.da, Xa), O::mul(w, O::mul(m.a, qu))), O::mul(w, O::mul(ceq, O::add(both(1.0f), qu))));
@@ -481,8 +482,11 @@ __device__ __forceinline__ void paired_step_node(const StepArgs &a, Geo &g, bool
         oa[2] = O::fma(aw, vc, x);
         ob[2] = O::fnma(aw, vc, x);
       }
-      // (the order of the stores: D2Q9 79.5 us a step of the 2D box this way
-      // and 84.3 the other, D3Q19 FP32 1.40 ms at 256 x 256 x 128 and 1.47)
+      // (The order of the stores, the same bits either way: D2Q9, at 96
+      // registers, 79.5 us a step of the 2D box this way and 84.3 the other, D3Q19
+      // FP32, at 168, 1.40 ms at 256 x 256 x 128 this way and 1.47 the other.  Like
+      // the grouping above it is the register allocation's choice, to be measured
+      // again when the launch bounds or the compiler change.)
       if (Q == 19) {
         finish(qo, ob, INTc);
         finish(q, oa, INTc);
